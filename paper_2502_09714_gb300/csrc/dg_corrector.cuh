@@ -5,6 +5,7 @@
 #include <type_traits>
 
 #include "dg_sparse.cuh"
+#include "dg_team.h"
 
 namespace dg {
 
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
   extern __shared__ float4 smem4[];
   __shared__ __align__(8) uint64_t mbars[C::TEAMS];
   __shared__ uint32_t tmem_base;
-  __shared__ volatile int sStop[C::TEAMS];
+  __shared__ TeamStop stops[C::TEAMS];
   const float* tb = a.tables;
   const float dt = a.dt;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
   if (warp == 0) tc::alloc(&tmem_base, C::TMEM_COLS);
   if (threadIdx.x < C::TEAMS) {
     tc::mbar_init(&mbars[threadIdx.x], 1);
-    sStop[threadIdx.x] = 0;
+    stops[threadIdx.x].init();
   }
   tc::fence_before();
   __syncthreads();
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
   const int bar_mma = 1 + team, bar_copy = 3 + team, bar_work = 5 + team;
   float* sm = reinterpret_cast<float*>(smem4) + team * C::TEAM_SMEM;
   uint64_t* mbar = &mbars[team];
+  TeamStop& stop = stops[team];
   const uint32_t dcol = tmem + team * C::DC;
   float* sBvH = sm + C::oOp;
   float* sBvL = sBvH + C::BV;
@@ -244,16 +246,16 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
     for (int it = 0;; tile += step, ++it) {
       tc::cp_async_wait_all();                 // this tile's copies have landed
       tc::named_barrier(bar_copy, C::TEAM_THREADS);   // the workers start on it; the other buffer is free
-      if (sStop[team]) break;
+      if (stop.copy_stops(it)) break;
       if (tile + step < ntiles)
         issue(tile + step, sm + C::oBuf + ((it + 1) & 1) * C::BUF,
               reinterpret_cast<const int*>(sm + C::oBuf + (it & 1) * C::BUF + C::bI));
     }
   } else if (warp >= MMA0) {
     // volume MMAs, then projection MMAs, each batch when the workers' operand is ready
-    for (;;) {
+    for (int n = 0;; n += 2) {
       tc::named_barrier(bar_mma, C::TEAM_THREADS);
-      if (sStop[team]) break;
+      if (stop.mma_stops(n)) break;
       if (lane == 0) {
         tc::fence_after();
         constexpr uint32_t id0 = tc::idesc_tf32(128, N0), idh = tc::idesc_tf32(128, NH);
@@ -278,7 +280,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
       }
       __syncwarp();
       tc::named_barrier(bar_mma, C::TEAM_THREADS);
-      if (sStop[team]) break;
+      if (stop.mma_stops(n + 1)) break;
       if (lane == 0) {
         tc::fence_after();
         constexpr uint32_t idp = tc::idesc_tf32(128, NPC);
@@ -429,6 +431,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
         const bool ok = tc::wait_parity(mbar, phase, wait_limit);
         phase ^= 1u;
         if (tc::named_barrier_or(bar_work, C::WORKERS, !ok)) {
+          if (tid == 0) stop.set(it, 1);
           failed = true;
           break;
         }
@@ -515,6 +518,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
         const bool ok = tc::wait_parity(mbar, phase, wait_limit);
         phase ^= 1u;
         if (tc::named_barrier_or(bar_work, C::WORKERS, !ok)) {
+          if (tid == 0) stop.set(it, 2);
           failed = true;
           break;
         }
@@ -580,7 +584,7 @@ __global__ void __launch_bounds__(CorrTcCfg<N, TILE>::THREADS, 1) k_corrector_tc
       if (tid == 0) atomicOr(a.status, kStatusTimeout);
       tc::wait_parity(mbar, phase ^ 1u, kWaitLimit);   // let the MMAs in flight finish before freeing TMEM
     }
-    if (tid == 0) sStop[team] = 1;
+    if (tid == 0 && !failed) stop.set(it, 0);
     __threadfence_block();
     tc::named_barrier(bar_mma, C::TEAM_THREADS);       // releases the MMA warp
     tc::named_barrier(bar_copy, C::TEAM_THREADS);      // and the copy warp
