@@ -71,11 +71,9 @@ typedef enum {
 /* Optional device allocator (e.g. a framework's caching allocator).  alloc must
  * return a device pointer aligned to at least 256 bytes, or NULL on failure.
  * NULL in dg_mesh_desc.alloc selects cudaMalloc/cudaFree.
- * One buffer of a context is optional: the elements' modal traces on their faces
- * (4.7 KB per element copy at N = 4), requested by dg_mesh_create when at least as
- * much device memory stays free.  Without it the face kernel takes its own traces
- * (the same states bit for bit, slower).  When a later request is refused, the
- * library frees it and asks again. */
+ * One buffer is optional and never held between calls: the elements' modal traces on
+ * their faces (see dg_set_modal_traces), requested at the start of a call and given
+ * back at its end; a refusal is no error. */
 typedef struct {
   void* (*alloc)(size_t bytes, void* stream, void* user);
   void (*free)(void* ptr, size_t bytes, void* stream, void* user);
@@ -153,6 +151,21 @@ dg_status dg_set_predictor(dg_ctx* ctx, int kind, int iterations);
  * is how the failure path is tested without any fault.  Not a passage of the
  * paper: the waits belong to this library's kernels.  DG_E_ARG above 2^31 - 1. */
 dg_status dg_set_wait_limit(dg_ctx* ctx, int64_t polls);
+
+/* Device memory for the elements' modal traces on their faces (4.7 KB per element copy at
+ * N = 4), which dg_step, dg_step_host and dg_adjoint_gradient take for the duration of the
+ * call: with them the predictor hands the traces to the face kernel, without them the face
+ * kernel takes its own (the same states bit for bit, slower; the Picard predictor,
+ * dg_step_noalloc and small meshes of degree 5 never take them).  max_bytes < 0, the
+ * default: taken where at least as much device memory stays free.  max_bytes >= 0: taken up
+ * to that size whatever is free; 0 never.  Without a dg_mesh_desc.alloc the memory comes from
+ * a stream-ordered pool of the context, which keeps it between calls: cudaMemGetInfo counts
+ * it as used, and the driver returns it to any other allocation of the process that would
+ * fail otherwise.  This call returns what the pool keeps, and dg_destroy the rest.
+ * dg_modal_trace_bytes: the size that the last of those calls ran with, 0 without traces.
+ * Not a passage of the paper. */
+dg_status dg_set_modal_traces(dg_ctx* ctx, int64_t max_bytes);
+int64_t dg_modal_trace_bytes(const dg_ctx* ctx);
 
 /* Per-element material [n_elem][6] = (rho, lambda0, mu0, gamma_r, xi0, C_d):
  * density, Lame parameters of the intact rock, damage modulus gamma_r [Pa],

@@ -108,7 +108,12 @@ struct dg_ctx {
   float* d = nullptr;
   float* cp = nullptr;
   float* ff = nullptr;               // face fluxes
-  float* tr = nullptr;               // modal traces from the predictor, when memory allows
+  // modal traces from the predictor: held during a call only, when memory allows
+  float* tr = nullptr;
+  int64_t tr_limit = -1;             // dg_set_modal_traces
+  int64_t tr_bytes = 0;              // of the last call
+  bool tr_granted = false;           // the allocator gave them to the last call that asked
+  cudaMemPool_t tr_pool = nullptr;   // their memory between calls (without an allocator of the caller's)
   int4* faces = nullptr;
   int* elem_face = nullptr;
   int64_t F = 0;            // faces in the flux list: interior first, then boundary
@@ -187,35 +192,96 @@ void* dev_try_alloc(dg_ctx* ctx, size_t bytes) {
   return p;
 }
 
-void* dev_alloc(dg_ctx* ctx, size_t bytes) {
-  if (bytes == 0) bytes = 16;
-  void* p = nullptr;
-  for (;;) {
-    p = dev_try_alloc(ctx, bytes);
-    if (p || !ctx->tr) break;
-    // the modal traces are optional (without them the face kernel takes its own): give them back
+// Gives the modal traces back: to the caller's allocator (which may hand them to another stream, hence the wait
+// before), or to the context's pool (whose memory the driver returns to others once a wait has seen it freed).
+void drop_traces(dg_ctx* ctx) {
+  if (!ctx->tr) return;
+  if (ctx->has_alloc) {
     cudaStreamSynchronize(ctx->stream);
     dev_free(ctx, ctx->tr);
-    ctx->tr = nullptr;
+  } else {
+    cudaFreeAsync(ctx->tr, ctx->stream);
+    cudaStreamSynchronize(ctx->stream);
+  }
+  ctx->tr = nullptr;
+}
+
+void* dev_alloc(dg_ctx* ctx, size_t bytes) {
+  if (bytes == 0) bytes = 16;
+  void* p = dev_try_alloc(ctx, bytes);
+  if (!p && ctx->tr) {
+    // the modal traces are optional (without them the face kernel takes its own): give them back
+    drop_traces(ctx);
+    ctx->tr_bytes = 0;
+    if (ctx->tr_pool) cudaMemPoolTrimTo(ctx->tr_pool, 0);
+    p = dev_try_alloc(ctx, bytes);
   }
   return p;
 }
 
-// Room for the modal traces, [E][4][tr_stride] floats: taken when it leaves at least as much
-// device memory free as it uses, so that a mesh near the device's capacity runs as without it.  Degree 5, whose
-// predictor stages one face at a time, takes it from one round of the predictor's CTAs on (two per SM, 16
-// elements each): predictor and faces 331 -> 288 us on 16,464 tets and 139 -> 128 us on 6,000, but 35 -> 40 us
-// on 384.
+// Room for the modal traces, [E][4][tr_stride] floats: taken when it leaves at least as much device memory free as
+// it uses (or up to the limit of dg_set_modal_traces).  Degree 5, whose predictor stages one face at a time, takes it
+// from one round of the predictor's CTAs on (two per SM, 16 elements each): predictor and faces 331 -> 288 us on
+// 16,464 tets and 139 -> 128 us on 6,000, but 35 -> 40 us on 384.
+//
+// It is held for one call: what fits on the device beside a context is the same as without it.  Between calls the
+// memory stays in a pool of the context, from which the driver returns it to any other allocation of the process
+// that would fail (180 GiB by cudaMalloc beside 120 kept ones); taking it from there and giving it back costs 3 us,
+// cudaMalloc and cudaFree 95 us for 64 MiB and 840 us for 1 GiB.
 void take_traces(dg_ctx* ctx) {
+  ctx->tr_bytes = 0;
+  if (ctx->picard_iters > 0) return;            // the Picard iterations change the predictor's output
   if (ctx->N == 5 && ctx->EV < static_cast<int64_t>(2) * 16 * ctx->grid_pred) return;
   const size_t bytes = sizeof(float) * 4 * static_cast<size_t>(tr_stride(ctx->N)) * static_cast<size_t>(ctx->EV);
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-    cudaGetLastError();
-    return;
+  if (ctx->tr_limit >= 0 && bytes > static_cast<size_t>(ctx->tr_limit)) return;
+  if (!ctx->has_alloc && !ctx->tr_pool) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    uint64_t keep = UINT64_MAX;
+    if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&ctx->tr_pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(ctx->tr_pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      if (ctx->tr_pool) cudaMemPoolDestroy(ctx->tr_pool);
+      ctx->tr_pool = nullptr;
+      return;
+    }
   }
-  if (bytes <= free_b / 2) ctx->tr = static_cast<float*>(dev_alloc(ctx, bytes));
+  // what the pool still holds, or the allocator gave to the last call, is asked for again without the rule
+  bool ask = ctx->tr_limit >= 0 || ctx->tr_granted;
+  if (!ctx->has_alloc && !ask) {
+    uint64_t held = 0;
+    ask = cudaMemPoolGetAttribute(ctx->tr_pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess && held >= bytes;
+  }
+  if (!ask) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+    ask = bytes <= free_b / 2;
+  }
+  if (!ask) return;
+  if (ctx->has_alloc) {
+    ctx->tr = static_cast<float*>(dev_try_alloc(ctx, bytes));
+    ctx->tr_granted = ctx->tr != nullptr;
+  } else {
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, bytes, ctx->tr_pool, ctx->stream) == cudaSuccess) {
+      ctx->tr = static_cast<float*>(p);
+    } else {
+      cudaGetLastError();
+      cudaMemPoolTrimTo(ctx->tr_pool, 0);       // a refused request may leave memory in the pool
+    }
+  }
+  if (ctx->tr) ctx->tr_bytes = static_cast<int64_t>(bytes);
 }
+
+// The modal traces of one call, on every path out of it.
+struct TraceRoom {
+  dg_ctx* ctx;
+  explicit TraceRoom(dg_ctx* c) : ctx(c) { take_traces(c); }
+  ~TraceRoom() { drop_traces(ctx); }
+  TraceRoom(const TraceRoom&) = delete;
+  TraceRoom& operator=(const TraceRoom&) = delete;
+};
 
 void dev_free(dg_ctx* ctx, void* p) {
   if (!p) return;
@@ -521,6 +587,7 @@ void dg_destroy(dg_ctx* ctx) {
   for (cudaEvent_t ev : ctx->events) cudaEventDestroy(ev);
   for (cudaEvent_t ev : ctx->xfer_events) cudaEventDestroy(ev);
   if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+  if (ctx->tr_pool) cudaMemPoolDestroy(ctx->tr_pool);
   delete ctx;
 }
 
@@ -780,7 +847,6 @@ dg_status dg_mesh_create(const dg_mesh_desc* desc, dg_ctx** out) {
     }
     cudaGetLastError();
   }
-  take_traces(ctx);
   *out = ctx;
   return DG_OK;
 }
@@ -797,6 +863,16 @@ dg_status dg_set_predictor(dg_ctx* ctx, int kind, int iterations) {
   ctx->picard_iters = iterations;
   return DG_OK;
 }
+
+dg_status dg_set_modal_traces(dg_ctx* ctx, int64_t max_bytes) {
+  if (!ctx) return fail(ctx, DG_E_ARG, "NULL context");
+  ctx->tr_limit = max_bytes < 0 ? -1 : max_bytes;
+  ctx->tr_granted = false;
+  if (ctx->tr_pool) DG_CUDA(ctx, cudaMemPoolTrimTo(ctx->tr_pool, 0));
+  return DG_OK;
+}
+
+int64_t dg_modal_trace_bytes(const dg_ctx* ctx) { return ctx ? ctx->tr_bytes : 0; }
 
 dg_status dg_set_wait_limit(dg_ctx* ctx, int64_t polls) {
   if (!ctx) return fail(ctx, DG_E_ARG, "NULL context");
@@ -1096,6 +1172,7 @@ dg_status dg_step(dg_ctx* ctx, int64_t n_steps, double dt) {
     dg_status st = prepare_steps(ctx, n_steps, dt);
     if (st != DG_OK) return st;
   }
+  TraceRoom room(ctx);
   DG_CUDA(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned), ctx->stream));
   // events for per-kernel timing
   const int per_step = 3 + (nsrc > 0) + (R > 0);
@@ -1121,7 +1198,7 @@ dg_status dg_step(dg_ctx* ctx, int64_t n_steps, double dt) {
   a.d = ctx->d;
   a.cp = ctx->cp;
   a.ff = ctx->ff;
-  a.tr = ctx->picard_iters > 0 ? nullptr : ctx->tr;   // the Picard iterations change the predictor's output
+  a.tr = ctx->tr;
   a.faces = ctx->faces;
   a.elem_face = ctx->elem_face;
   a.grid_pred = ctx->grid_pred;
@@ -1222,6 +1299,7 @@ dg_status dg_step_host(dg_ctx* ctx, const float* q_in, float* q_out, double dt) 
     dg_status st = ensure_staging(ctx, sizeof(float) * row * E);
     if (st != DG_OK) return st;
   }
+  TraceRoom room(ctx);
   const std::vector<int64_t> cb = host_chunk_bounds(E);
   const int C = static_cast<int>(cb.size()) - 1;
   const bool face_ranges = ctx->host_faces.size() == static_cast<size_t>(C);
@@ -1247,7 +1325,7 @@ dg_status dg_step_host(dg_ctx* ctx, const float* q_in, float* q_out, double dt) 
   a.d = ctx->d;
   a.cp = ctx->cp;
   a.ff = ctx->ff;
-  a.tr = ctx->picard_iters > 0 ? nullptr : ctx->tr;   // the Picard iterations change the predictor's output
+  a.tr = ctx->tr;
   a.faces = ctx->faces;
   a.elem_face = ctx->elem_face;
   a.grid_pred = ctx->grid_pred;
@@ -1385,6 +1463,7 @@ dg_status dg_adjoint_gradient(dg_ctx* ctx, int64_t n_steps, double dt, const flo
   if (R < 1) return fail(ctx, DG_E_STATE, "the misfit needs receivers (dg_receivers)");
   if (dt <= 0) dt = ctx->dt_cfl;
   if (!std::isfinite(dt)) return fail(ctx, DG_E_ARG, "non-finite dt");
+  TraceRoom room(ctx);
   if (snapshots == 0) {
     // as many state copies as 80 % of the free device memory holds beside the call's other
     // buffers, at most the whole history
@@ -1478,7 +1557,7 @@ dg_status dg_adjoint_gradient(dg_ctx* ctx, int64_t n_steps, double dt, const flo
   a.d = ctx->d;
   a.cp = ctx->cp;
   a.ff = ctx->ff;
-  a.tr = ctx->picard_iters > 0 ? nullptr : ctx->tr;   // the Picard iterations change the predictor's output
+  a.tr = ctx->tr;
   a.faces = ctx->faces;
   a.elem_face = ctx->elem_face;
   a.grid_pred = ctx->grid_pred;

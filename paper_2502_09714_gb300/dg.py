@@ -25,7 +25,8 @@ EXPORTS = (
     "dg_receivers", "dg_receivers_read", "dg_dt", "dg_time", "dg_n_modes", "dg_get_stats",
     "dg_profile_enable", "dg_profile_read", "dg_reference_table", "dg_last_error", "dg_destroy",
     "dg_step_noalloc", "dg_set_rheology", "dg_set_predictor", "dg_set_wait_limit", "dg_step_host",
-    "dg_adjoint_gradient", "dg_revolve_plan", "dg_revolve_cost", "dg_host_chunks",
+    "dg_adjoint_gradient", "dg_revolve_plan", "dg_revolve_cost", "dg_host_chunks", "dg_set_modal_traces",
+    "dg_modal_trace_bytes",
 )
 
 
@@ -88,6 +89,8 @@ def load_library(path: str | None = None) -> C.CDLL:
         "dg_set_rheology": ([vp, C.c_int], C.c_int),
         "dg_set_predictor": ([vp, C.c_int, C.c_int], C.c_int),
         "dg_set_wait_limit": ([vp, i64], C.c_int),
+        "dg_set_modal_traces": ([vp, i64], C.c_int),
+        "dg_modal_trace_bytes": ([vp], i64),
         "dg_step_host": ([vp, vp, vp, C.c_double], C.c_int),
         "dg_host_chunks": ([i64, vp, C.c_int], C.c_int),
         "dg_set_source": ([vp, C.POINTER(PointSource), i64], C.c_int),
@@ -236,6 +239,16 @@ class Solver:
     def set_wait_limit(self, polls=-1):
         """Polls per bounded wait of the tensor-core corrector (negative: default)."""
         self._chk(self.lib.dg_set_wait_limit(self.ctx, int(polls)))
+
+    def set_modal_traces(self, max_bytes=-1):
+        """Limit of the device memory that a step takes for the modal traces during the call
+        (negative: half of what is free, the default; 0: none)."""
+        self._chk(self.lib.dg_set_modal_traces(self.ctx, int(max_bytes)))
+
+    @property
+    def modal_trace_bytes(self):
+        """Size of the modal traces that the last step ran with (0: without them)."""
+        return self.lib.dg_modal_trace_bytes(self.ctx)
 
     # ------------------------------------------------------------------
     def _chk(self, status):
