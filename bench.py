@@ -766,19 +766,24 @@ def _kernel_name(kind, N):
     return f"{names.get(kind, 'k_' + kind)}<{N}, 0>"
 
 
-def _kernel_source_digest():
-    """Digest of the step kernels' code: comments and spacing are left out, so that
-    a change of wording keeps the DRAM counters taken on the same code."""
+def _kernel_source_digest(csrc=os.path.join(ROOT, "paper_2502_09714_gb300", "csrc")):
+    """Digest of the step kernels' code, every file that they include (the generated lists of the
+    basis by their generator): comments and spacing are left out, so that a change of wording
+    keeps the DRAM counters taken on the same code."""
     import hashlib
     import re
-    h = hashlib.sha256()
-    for name in ("dg_step_kernels.cuh", "dg_predictor.cuh", "dg_faces.cuh", "dg_corrector.cuh", "dg_sparse.cuh"):
-        with open(os.path.join(ROOT, "paper_2502_09714_gb300", "csrc", name), encoding="utf-8") as f:
+    files, code = ["dg_step_kernels.cuh"], []
+    for name in files:
+        with open(os.path.join(csrc, name), encoding="utf-8") as f:
             src = f.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
         src = re.sub(r"//[^\n]*", " ", src)
-        h.update(" ".join(src.split()).encode())
-    return h.hexdigest()[:16]
+        code.append(" ".join(src.split()))
+        for inc in re.findall(r'#include "([^"]+)"', src):
+            new = ["gen/basis_lists.cpp", "dg_reference.cpp"] if inc == "dg_basis_lists.h" else \
+                [os.path.normpath(os.path.join(os.path.dirname(name), inc))]
+            files += [n for n in new if n not in files]
+    return hashlib.sha256("\n".join(code).encode()).hexdigest()[:16]
 
 
 def _traffic_per_launch(kernel, N, E):
