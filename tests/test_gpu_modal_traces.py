@@ -5,8 +5,11 @@ import pytest
 
 from oracle import to_abi
 from synthetic import periodic_cube_mesh, rock_material
+from synthetic.mesh import FACE_BC_ABSORBING, FACE_BC_FREE_SURFACE
 
-from test_gpu_boundary import _rough_state
+from parity_util import make_solver
+from test_gpu_boundary import _box, _rough_state
+from test_gpu_picard import _material
 
 pytestmark = pytest.mark.gpu
 
@@ -149,4 +152,35 @@ def test_other_allocations_get_the_kept_memory():
     torch.cuda.empty_cache()
     s.step(1, 0.5 * s.dt)                               # and the traces are there again
     assert s.modal_trace_bytes > 100e6
+    s.close()
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5])
+def test_both_paths_with_boundaries_over_several_rounds(N):
+    """5,400 tets with outer faces, above the size from which degree 5 takes the traces (one face staged at a time):
+    the whole state with and without them."""
+    import torch
+    mesh = _box((10, 10, 9), (False, False, False), FACE_BC_FREE_SURFACE, FACE_BC_ABSORBING, seed=N)
+    least = 32 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert mesh.n_elem >= least
+    mat = _material("cdm", mesh.n_elem, np.random.default_rng(N))
+    Q = to_abi(_rough_state(mesh.n_elem, N, seed=N))
+    s = make_solver(mesh, mat, N)
+    q = _step(s, Q)
+    assert s.modal_trace_bytes > 0
+    s.set_modal_traces(0)
+    np.testing.assert_array_equal(_step(s, Q), q)
+    assert s.modal_trace_bytes == 0
+    assert np.isfinite(q).all() and np.abs(q - Q).max() > 0
+    s.close()
+
+
+def test_small_meshes_of_degree_5_run_without():
+    mesh, mat, Q = _problem(5)
+    s = _solver(mesh, mat, 5)
+    _step(s, Q)
+    assert s.modal_trace_bytes == 0
+    s.set_modal_traces(1 << 40)
+    _step(s, Q)
+    assert s.modal_trace_bytes == 0
     s.close()
