@@ -1351,7 +1351,7 @@ dg_status dg_step_host(dg_ctx* ctx, const float* q_in, float* q_out, double dt) 
     if (a.tr) c.tr = a.tr + e0 * 4 * tr_stride(ctx->N);
     c.geom = a.geom + e0;
     c.mat = a.mat + e0;
-      c.elem_face = a.elem_face + e0 * 4;
+    c.elem_face = a.elem_face + e0 * 4;
     return c;
   };
   DG_CUDA(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned), ctx->stream));

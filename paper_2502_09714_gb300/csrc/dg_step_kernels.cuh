@@ -23,7 +23,6 @@
 #pragma once
 
 #include <algorithm>
-#include <cstdlib>
 
 #include "dg_internal.h"
 #include "dg_tc.cuh"
@@ -174,17 +173,7 @@ __device__ __forceinline__ void boundary_flux(int bc, const float u[9], const fl
 }  // namespace dg
 
 #include "dg_predictor.cuh"
-
-namespace dg {
-
-}  // namespace dg
-
 #include "dg_faces.cuh"
-
-namespace dg {
-
-}  // namespace dg
-
 #include "dg_corrector.cuh"
 #include "dg_planes.cuh"
 
@@ -193,36 +182,15 @@ namespace dg {
 // ---------------------------------------------------------------------------
 template <class Cfg, class Kern>
 cudaError_t launch_persistent(Kern kern, int64_t tiles, int grid_hint, const StepArgs& a, cudaStream_t s,
-                              bool* configured, int* max_blocks, int cap_per_sm = 0) {
+                              bool* configured, int* max_blocks, int per_sm = 0) {
   const size_t smem = sizeof(float) * Cfg::SMEM;
   if (!*configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if (cap_per_sm > 0) {
-      // Kernels holding tensor memory: the occupancy query counts one block per SM for any
-      // kernel that allocates it, whatever it allocates.  The blocks that shared memory,
-      // registers and threads allow are resident; of those, cap_per_sm fit in the SM's
-      // 512 columns (a block that finds too few waits in its allocation, it cannot deadlock).
-      cudaFuncAttributes fa{};
-      e = cudaFuncGetAttributes(&fa, kern);
-      if (e != cudaSuccess) return e;
-      int dev = 0, sm_smem = 0, reserved = 0, sm_regs = 0, sm_threads = 0;
-      if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-          (e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess ||
-          (e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess ||
-          (e = cudaDeviceGetAttribute(&sm_regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev)) != cudaSuccess ||
-          (e = cudaDeviceGetAttribute(&sm_threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev)) != cudaSuccess)
-        return e;
-      const int warps = (Cfg::THREADS + 31) / 32;
-      const int regs_warp = (fa.numRegs * 32 + 255) / 256 * 256;      // allocated per warp in units of 256
-      const int by_smem = static_cast<int>(static_cast<size_t>(sm_smem) / (smem + fa.sharedSizeBytes + reserved));
-      const int by_regs = regs_warp > 0 ? sm_regs / (regs_warp * warps) : cap_per_sm;
-      const int by_threads = sm_threads / Cfg::THREADS;
-      per_sm = std::min(std::min(by_smem, by_regs), std::min(by_threads, cap_per_sm));
-    } else {
+    // per_sm given: kernels holding tensor memory, for which the occupancy query does not count by its columns
+    if (per_sm == 0) {
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Cfg::THREADS, smem);
       if (e != cudaSuccess) return e;
     }
