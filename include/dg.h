@@ -159,9 +159,10 @@ dg_status dg_set_wait_limit(dg_ctx* ctx, int64_t polls);
  * dg_step_noalloc and small meshes of degree 5 never take them).  max_bytes < 0, the
  * default: taken where at least as much device memory stays free.  max_bytes >= 0: taken up
  * to that size whatever is free; 0 never.  Without a dg_mesh_desc.alloc the memory comes from
- * a stream-ordered pool of the context, which keeps it between calls: cudaMemGetInfo counts
- * it as used, and the driver returns it to any other allocation of the process that would
- * fail otherwise.  This call returns what the pool keeps, and dg_destroy the rest.
+ * a stream-ordered pool of the context, filled by dg_mesh_create, which keeps it between calls:
+ * cudaMemGetInfo counts it as used, and the driver returns it to any other allocation of the
+ * process that would fail otherwise.  This call returns what the pool keeps (as does choosing
+ * the Picard predictor), and dg_destroy the rest.
  * dg_modal_trace_bytes: the size that the last of those calls ran with, 0 without traces.
  * Not a passage of the paper. */
 dg_status dg_set_modal_traces(dg_ctx* ctx, int64_t max_bytes);
