@@ -38,7 +38,7 @@ namespace dg {
 // Bound by instruction issue and latency: a team's tile takes 18.6k cycles at degree 4 (operand 2.3k,
 // lift and strain rows 2.9k, law 5.3k, read-out and velocity rows 2.8k, update 1.5k, waits on the MMAs
 // 3.2k), with both teams in flight.  Against one team of 15 workers on nodal-time columns, dense modal
-// derivatives and three MMAs per K step of the projection: 2.21 -> 1.37 ms on the 196,608-tet cube of
+// derivatives and three MMAs per K step of the projection: 2.21 -> 1.35 ms on the 196,608-tet cube of
 // degree 4, 2.57 -> 1.31 ms on 331,776 element copies of degree 3, 45 -> 23 us on 5,184 tets of degree 2.
 // Tiles of eight elements at degree 3, which spread the barriers, the waits and the velocity rows (24 lanes of a
 // warp in place of 12) over twice the work: 1.31 -> 1.02 ms.
