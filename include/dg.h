@@ -71,7 +71,7 @@ typedef enum {
 /* Optional device allocator (e.g. a framework's caching allocator).  alloc must
  * return a device pointer aligned to at least 256 bytes, or NULL on failure.
  * NULL in dg_mesh_desc.alloc selects cudaMalloc/cudaFree.
- * One buffer is optional and never held between calls: the elements' modal traces on
+ * One buffer is optional and not held between calls: the elements' modal traces on
  * their faces (see dg_set_modal_traces), requested at the start of a call and given
  * back at its end; a refusal is no error. */
 typedef struct {
@@ -161,8 +161,8 @@ dg_status dg_set_wait_limit(dg_ctx* ctx, int64_t polls);
  * to that size whatever is free; 0 never.  Without a dg_mesh_desc.alloc the memory comes from
  * a stream-ordered pool of the context, filled by dg_mesh_create, which keeps it between calls:
  * cudaMemGetInfo counts it as used, and the driver returns it to any other allocation of the
- * process that would fail otherwise.  This call returns what the pool keeps (as does choosing
- * the Picard predictor), and dg_destroy the rest.
+ * process that would fail otherwise; up to 2 MiB are a buffer that the context keeps.  This call
+ * returns what is kept (as does choosing the Picard predictor), and dg_destroy the rest.
  * dg_modal_trace_bytes: the size that the last of those calls ran with, 0 without traces.
  * Not a passage of the paper. */
 dg_status dg_set_modal_traces(dg_ctx* ctx, int64_t max_bytes);

@@ -113,7 +113,8 @@ struct dg_ctx {
   int64_t tr_limit = -1;             // dg_set_modal_traces
   int64_t tr_bytes = 0;              // of the last call
   bool tr_granted = false;           // the last call that asked got them
-  cudaMemPool_t tr_pool = nullptr;   // their memory between calls (without an allocator of the caller's)
+  cudaMemPool_t tr_pool = nullptr;   // their memory between calls (without an allocator of the caller's),
+  float* tr_kept = nullptr;          //   or, small ones, a buffer that the context keeps
   int4* faces = nullptr;
   int* elem_face = nullptr;
   int64_t F = 0;            // faces in the flux list: interior first, then boundary
@@ -196,6 +197,10 @@ void* dev_try_alloc(dg_ctx* ctx, size_t bytes) {
 // before), or to the context's pool (whose memory the driver returns to others once a wait has seen it freed).
 void drop_traces(dg_ctx* ctx) {
   if (!ctx->tr) return;
+  if (ctx->tr == ctx->tr_kept) {
+    ctx->tr = nullptr;
+    return;
+  }
   if (ctx->has_alloc) {
     cudaStreamSynchronize(ctx->stream);
     dev_free(ctx, ctx->tr);
@@ -206,14 +211,25 @@ void drop_traces(dg_ctx* ctx) {
   ctx->tr = nullptr;
 }
 
+// And what the context keeps of their memory between calls.
+void free_traces(dg_ctx* ctx) {
+  drop_traces(ctx);
+  ctx->tr_granted = false;
+  if (ctx->tr_kept) {
+    cudaStreamSynchronize(ctx->stream);
+    dev_free(ctx, ctx->tr_kept);
+    ctx->tr_kept = nullptr;
+  }
+  if (ctx->tr_pool && cudaMemPoolTrimTo(ctx->tr_pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
 void* dev_alloc(dg_ctx* ctx, size_t bytes) {
   if (bytes == 0) bytes = 16;
   void* p = dev_try_alloc(ctx, bytes);
-  if (!p && ctx->tr) {
+  if (!p && (ctx->tr || ctx->tr_kept)) {
     // the modal traces are optional (without them the face kernel takes its own): give them back
-    drop_traces(ctx);
+    free_traces(ctx);
     ctx->tr_bytes = 0;
-    if (ctx->tr_pool) cudaMemPoolTrimTo(ctx->tr_pool, 0);
     p = dev_try_alloc(ctx, bytes);
   }
   return p;
@@ -227,14 +243,23 @@ void* dev_alloc(dg_ctx* ctx, size_t bytes) {
 // It is held for one call: what fits on the device beside a context is the same as without it.  Between calls the
 // memory stays in a pool of the context, from which the driver returns it to any other allocation of the process
 // that would fail (180 GiB by cudaMalloc beside 120 kept ones); taking it from there and giving it back costs 3 us,
-// cudaMalloc and cudaFree 95 us for 64 MiB and 840 us for 1 GiB.
+// cudaMalloc and cudaFree 95 us for 64 MiB and 840 us for 1 GiB.  Up to the 2 MiB in which the driver maps memory
+// (1,400 tets at degree 2, 440 at degree 4) the context keeps a plain buffer instead: creating a pool takes 0.3 ms of
+// dg_mesh_create, and it maps 32 MiB at least (20 steps of 384 tets of degree 2: 348 us, 351 with a pool).
+constexpr size_t kKeptTraces = size_t(2) << 20;
 void take_traces(dg_ctx* ctx) {
   ctx->tr_bytes = 0;
   if (ctx->picard_iters > 0) return;            // the Picard iterations change the predictor's output
   if (ctx->N == 5 && ctx->EV < static_cast<int64_t>(2) * 16 * ctx->grid_pred) return;
   const size_t bytes = sizeof(float) * 4 * static_cast<size_t>(tr_stride(ctx->N)) * static_cast<size_t>(ctx->EV);
   if (ctx->tr_limit >= 0 && bytes > static_cast<size_t>(ctx->tr_limit)) return;
-  if (!ctx->has_alloc && !ctx->tr_pool) {
+  if (ctx->tr_kept) {
+    ctx->tr = ctx->tr_kept;
+    ctx->tr_bytes = static_cast<int64_t>(bytes);
+    return;
+  }
+  const bool keep_it = !ctx->has_alloc && bytes <= kKeptTraces;
+  if (!ctx->has_alloc && !keep_it && !ctx->tr_pool) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -254,8 +279,9 @@ void take_traces(dg_ctx* ctx) {
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
     if (bytes > free_b / 2) return;
   }
-  if (ctx->has_alloc) {
+  if (ctx->has_alloc || keep_it) {
     ctx->tr = static_cast<float*>(dev_try_alloc(ctx, bytes));
+    if (keep_it) ctx->tr_kept = ctx->tr;
   } else {
     void* p = nullptr;
     if (cudaMallocFromPoolAsync(&p, bytes, ctx->tr_pool, ctx->stream) == cudaSuccess) {
@@ -276,7 +302,7 @@ struct TraceRoom {
   ~TraceRoom() { drop_traces(ctx); }
   void before_wait() {
     if (ctx->has_alloc || !ctx->tr) return;
-    cudaFreeAsync(ctx->tr, ctx->stream);
+    if (ctx->tr != ctx->tr_kept) cudaFreeAsync(ctx->tr, ctx->stream);
     ctx->tr = nullptr;
   }
   TraceRoom(const TraceRoom&) = delete;
@@ -847,7 +873,7 @@ dg_status dg_mesh_create(const dg_mesh_desc* desc, dg_ctx** out) {
     }
     cudaGetLastError();
   }
-  if (!ctx->has_alloc) {               // the pool's memory is there before the first step (0.2 ms of it for 384 tets)
+  if (!ctx->has_alloc) {               // the memory is there before the first step
     take_traces(ctx);
     drop_traces(ctx);
     ctx->tr_bytes = 0;
@@ -866,15 +892,14 @@ dg_status dg_set_predictor(dg_ctx* ctx, int kind, int iterations) {
     return fail(ctx, DG_E_ARG, "unknown predictor or iteration count");
   if (ctx->N > 4) return fail(ctx, DG_E_ORDER, "the Picard predictor supports degrees 1..4");
   ctx->picard_iters = iterations;
-  if (ctx->tr_pool) DG_CUDA(ctx, cudaMemPoolTrimTo(ctx->tr_pool, 0));   // it does without the modal traces
+  free_traces(ctx);                    // it does without them
   return DG_OK;
 }
 
 dg_status dg_set_modal_traces(dg_ctx* ctx, int64_t max_bytes) {
   if (!ctx) return fail(ctx, DG_E_ARG, "NULL context");
   ctx->tr_limit = max_bytes < 0 ? -1 : max_bytes;
-  ctx->tr_granted = false;
-  if (ctx->tr_pool) DG_CUDA(ctx, cudaMemPoolTrimTo(ctx->tr_pool, 0));
+  free_traces(ctx);
   return DG_OK;
 }
 
